@@ -257,9 +257,9 @@ emr_status emr_eval_chunk(const void *pack_host, const emr_query *q, const emr_g
 
 /* Filter a materialised evaluation (Section 3.2, Eq. 2; Theorem 1's band
  * threshold). out/out_halo as written by emr_eval. Writes three bit planes,
- * device uint32 [P * S][n_words] each: split (d < D and V > theta), band_bits
- * (B > band and the weight filter) and mask (emr_mask_combine of the two in
- * the given mode); var_dbg (optional, device float [P * S][n_total]) receives
+ * device uint32 [P * S][n_words] each, every word of them: split (d < D and
+ * V > theta; 0 at depth D), band_bits (B > band and the weight filter) and mask
+ * (emr_mask_combine of the two in the given mode); var_dbg (optional, device float [P * S][n_total]) receives
  * V(p). theta >= 0, band >= 0, w_min >= 0 (0 = weight filter off).
  * Errors: EMR_ERR_ARG, EMR_ERR_CUDA. */
 emr_status emr_variance_filter(const float *out, const float *out_halo, const emr_grid *grid, int32_t P,
@@ -299,9 +299,10 @@ emr_status emr_substrate_config(int32_t config, int32_t *types, int32_t *hidden_
  * each tile of positions evaluates its points and the ring of neighbours it
  * needs, takes each parent cell's variance from its four children in registers
  * and each position's band value from shared memory, and writes only the split
- * and band_bits planes (as emr_variance_filter) plus, when out is not NULL, the
- * CPPN output at positions whose band test passed (other entries of out are
- * left untouched). Follow with emr_mask_combine. ws: prepared by
+ * and band_bits planes (as emr_variance_filter, but the split words of depth D,
+ * which hold no split and which no call reads, are left untouched) plus, when out
+ * is not NULL, the CPPN output at positions whose band test passed (other entries
+ * of out are left untouched). Follow with emr_mask_combine. ws: prepared by
  * emr_eval_prepare. Errors: EMR_ERR_ARG, EMR_ERR_CAPACITY, EMR_ERR_RANGE,
  * EMR_ERR_CUDA. */
 emr_status emr_eval_filter(const void *pack_host, const emr_query *q, const emr_grid *grid, float theta,
