@@ -46,3 +46,17 @@ def test_every_word_is_written(D, mode):
     bits = unpack_planes(dirty[1].cpu().numpy(), g)
     clear = np.abs(v - 0.3) > tol
     assert np.array_equal(bits[clear], (v > 0.3)[clear])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("D", [0, 4, 5, 6])
+@pytest.mark.parametrize("offset", [1, 2, 3])
+def test_variances_at_any_float(D, offset):
+    """var_dbg may be a view that begins at any float of a larger buffer."""
+    n = 3
+    g, out, halo = _inputs(D, n)
+    dev = out.cuda(), halo.cuda()
+    _, want = _filter(g, *dev, n, emr.EMR_EAGER, 0)
+    _, got = _filter(g, *dev, n, emr.EMR_EAGER, 0, offset)
+    assert got.data_ptr() % 16 == 4 * offset
+    assert torch.equal(got, want)
