@@ -60,3 +60,19 @@ def test_variances_at_any_float(D, offset):
     _, got = _filter(g, *dev, n, emr.EMR_EAGER, 0, offset)
     assert got.data_ptr() % 16 == 4 * offset
     assert torch.equal(got, want)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind", ["x", "y", "diagonal"])
+def test_variance_of_two_values_is_rounded_once(kind):
+    """Cells whose children hold two values, two of each: V = (a - b)^2 / 4 from the fp32 difference, the square
+    rounded once and scaled by a power of two, at every depth."""
+    D, n = 6, 5
+    g = emr.grid_build(D)
+    gen = torch.Generator().manual_seed(3)
+    ab = torch.randn(n, g.n_total // 4, 2, generator=gen)
+    out = ab[..., {"x": [0, 1, 0, 1], "y": [0, 0, 1, 1], "diagonal": [0, 1, 1, 0]}[kind]].reshape(n, g.n_total)
+    _, var = _filter(g, out.cuda(), torch.zeros(n, g.n_halo, device="cuda"), n, emr.EMR_EAGER, 0)
+    t = ab[..., 0] - ab[..., 1]
+    lo = g.level_off[D]
+    assert torch.equal(var.cpu()[:, :lo], (0.25 * (t * t))[:, 1:])
