@@ -589,7 +589,9 @@ emr_status emr_assemble(const void *pack_host, const void *pack_dev, int32_t n_i
  * take, at once, the sigmoid 1 / (1 + e^-z) of z = the weighted sum of their
  * sources' previous values (the substrate network of an HyperNEAT-style
  * indirect encoding, Section 2; recurrent connections make the result depend
- * on steps). out[(g * K + k) * n_out + o] receives output o. max_hidden: the
+ * on steps). out[(g * K + k) * n_out + o] receives output o. A network (in
+ * which a pair of nodes is connected at most once) gives the same bits for a
+ * pattern whatever the other networks and patterns of the call. max_hidden: the
  * largest hidden-node count of a genome (sizes shared memory: the call fails
  * with EMR_ERR_RANGE when 8 (n_in + n_out + max_hidden) K bytes do not fit).
  * Errors: EMR_ERR_ARG, EMR_ERR_RANGE, EMR_ERR_CUDA. */

@@ -144,8 +144,9 @@ __device__ __forceinline__ void ann_step(const AnnArgs& A, const cg::cluster_gro
   }
 }
 
-// Network g by one CTA, or (CLUSTER) by the cluster, whose CTAs all call this.
-template <int V, int KC, int NT, bool CLUSTER>
+// Network g by one CTA, or (CLUSTER) by the cluster, whose CTAs all call this. MID: a CTA's network
+// may have more than kAnnClusterConns connections.
+template <int V, int KC, int NT, bool CLUSTER, bool MID>
 __device__ __forceinline__ void ann_network(const AnnArgs& A, const cg::cluster_group& cl, int64_t g, float* sm) {
   const int tid = threadIdx.x, K = A.K;
   const int32_t N = A.n_in + A.n_out + int32_t(A.node_off[g + 1] - A.node_off[g]);
@@ -198,9 +199,15 @@ __device__ __forceinline__ void ann_network(const AnnArgs& A, const cg::cluster_
   // its lanes at once, 4 at least, since a pass over the nodes costs more in latency than connections
   // (952 networks of up to 95 nodes and 4.7 K connections, 4 patterns, 5 steps: 67 us with a warp a node from 16
   // connections a node on, 8 lanes below; 35 so, before the larger of them left the clusters).
+  // The lanes set the order of a node's sum, so they follow from the network alone: its bits are the
+  // same in every call. Up to kAnnNoClusters connections, where the call's other networks decide between
+  // a CTA and a cluster, 8 in both (30 batches of 200 networks, the largest of 110 to 700 hidden nodes, 1 to 16
+  // patterns, 4 steps: 35.9 us in the mean, 36.8 with each kernel's own rule there).
   const int32_t nodes = n_hi - n_lo;
-  const bool wide = CLUSTER ? e_hi - e_lo >= kAnnWideDegree * nodes : nodes <= NT / 32;
-  const bool narrow = !CLUSTER && nodes > NT / 8;
+  const int32_t degree = C > kAnnNoClusters ? kAnnWideDegree : int32_t(kAnnNoClusters) + 1;  // (no node has as many)
+  const bool eight = MID && C > kAnnClusterConns;
+  const bool wide = CLUSTER ? e_hi - e_lo >= degree * nodes : !eight && nodes <= NT / 32;
+  const bool narrow = !CLUSTER && !eight && nodes > NT / 8;
   for (int32_t step = 0; step < A.steps; step++) {
     if (wide)
       ann_step<V, KC, 32, NT, CLUSTER>(A, cl, cur, nxt, in_beg, n_lo, n_hi, src, w);
@@ -248,31 +255,34 @@ __global__ void __launch_bounds__(kAnnThreads, 1024 / kAnnThreads) ann_large_ker
 #pragma unroll
       for (int i = 0; i < kRounds; i++) b = i == k ? big[i] : b;
       for (; b; b &= b - 1, n_big++)
-        if (n_big % n_cl == my) ann_network<V, KC, kAnnThreads, true>(A, cl, g0 + 32 * k + __ffs(b) - 1, sm);
+        if (n_big % n_cl == my) ann_network<V, KC, kAnnThreads, true, false>(A, cl, g0 + 32 * k + __ffs(b) - 1, sm);
     }
   }
 }
 
 // The other networks, a CTA each. Launched to overlap ann_large_kernel (they share no output);
 // the last CTA waits for it as it exits, so that this launch completes after it.
-template <int V, int KC>
+template <int V, int KC, bool MID>
 __global__ void __launch_bounds__(kAnnSmallThreads, 1024 / kAnnSmallThreads) ann_small_kernel(const AnnArgs A) {
   extern __shared__ __align__(16) float sm[];
   const int64_t g = blockIdx.x;
   const cg::cluster_group cl = cg::this_cluster();
   if (A.conn_off[g + 1] - A.conn_off[g] <= A.cluster_conns)
-    ann_network<V, KC, kAnnSmallThreads, false>(A, cl, g, sm);
+    ann_network<V, KC, kAnnSmallThreads, false, MID>(A, cl, g, sm);
   if (g == A.P - 1) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 template <int V, int KC>
 cudaError_t launch_ann(AnnArgs A, int64_t max_conns, size_t smem, int sms, cudaStream_t st) {
   cudaError_t e;
+  // (the variant for networks that stay off the clusters despite their connections: its rule, taken by
+  // all, made the others' steps slower, 21.5 -> 24.3 us for 200 networks and one pattern)
+  const auto small = max_conns > kAnnClusterConns && max_conns <= kAnnNoClusters ? ann_small_kernel<V, KC, true>
+                                                                                : ann_small_kernel<V, KC, false>;
   if (smem > 48 * 1024) {
     if ((e = cudaFuncSetAttribute(ann_large_kernel<V, KC>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem))) !=
             cudaSuccess ||
-        (e = cudaFuncSetAttribute(ann_small_kernel<V, KC>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem))) !=
-            cudaSuccess)
+        (e = cudaFuncSetAttribute(small, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem))) != cudaSuccess)
       return e;
   }
   const int64_t clusters = std::max<int64_t>(1, std::min<int64_t>(A.P, 2 * sms / kAnnCluster));
@@ -298,7 +308,7 @@ cudaError_t launch_ann(AnnArgs A, int64_t max_conns, size_t smem, int sms, cudaS
   cfg.blockDim = dim3(kAnnSmallThreads);
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
-  return cudaLaunchKernelEx(&cfg, ann_small_kernel<V, KC>, A);
+  return cudaLaunchKernelEx(&cfg, small, A);
 }
 
 }  // namespace

@@ -103,3 +103,34 @@ def test_lanes_and_clusters_at_their_lines(sizes, density):
         got = emr.ann_forward(nets, pat, 3).cpu().numpy()
         ref, err = _reference(nets, pat, 3)
         assert np.all(np.abs(got - ref) <= err + 1e-30)
+
+
+def _one(nets, g):
+    h, src, dst, w, t = nets.genome(g)
+    return emr.Networks(nets.n_in, nets.n_out, np.array([0, len(h)], np.int64), h, np.array([0, len(w)], np.int64), src,
+                        dst, w, t)
+
+
+def _joined(a, b):
+    cat = lambda f: np.concatenate([getattr(a, f), getattr(b, f)])
+    off = lambda f: np.concatenate([getattr(a, f), getattr(a, f)[-1] + getattr(b, f)[1:]])
+    return emr.Networks(a.n_in, a.n_out, off("node_off"), cat("hidden"), off("conn_off"), cat("src"), cat("dst"),
+                        cat("w"), cat("type"))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("K", [1, 4, 6])
+def test_a_network_gives_the_same_bits_in_any_batch(K):
+    """Each network alone, beside its neighbours, and beside one that sizes the call's buffers far above it:
+    connection counts on both sides of the one that takes a cluster, nodes on both sides of a lane count's."""
+    sizes = [6, 30, 60, 88, 92, 96, 100, 104, 112, 120, 126, 140]
+    nets = _networks(sizes, 0.95, 3, 2, seed=K)
+    pat = np.random.default_rng(K).normal(0, 1, (K, 3)).astype(np.float32)
+    every = emr.ann_forward(nets, pat, 3)
+    large = emr.ann_forward(_joined(nets, _networks([700], 0.1, 3, 2, seed=7)), pat, 3)
+    for g in range(len(sizes)):
+        alone = emr.ann_forward(_one(nets, g), pat, 3)[0]
+        assert torch.equal(alone, every[g]), sizes[g]
+        assert torch.equal(alone, large[g]), sizes[g]
+    for k in range(K):
+        assert torch.equal(emr.ann_forward(nets, pat[k:k + 1], 3)[:, 0], every[:, k]), k
