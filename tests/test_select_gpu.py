@@ -156,3 +156,32 @@ def test_every_pair_is_scheduled_once(P):
         part.run_discover()
         for (i, v), (j, u) in zip(part.lists(), lists[4 * g0:]):
             assert np.array_equal(i, j) and np.array_equal(v.view(np.uint32), u.view(np.uint32))
+
+
+@pytest.mark.parametrize("n", [4095, 4096, 4097, 3 * 4096 + 5, 524288, 524289, 1 << 20, 1300001])
+def test_compaction_of_many_pairs(n):
+    """Pairs on both sides of one CTA of the offsets' scan (4096 counts) and of 128 CTAs, from where each scans
+    several times 4096: four positions a pair, kept at random."""
+    g = emr.grid_build(0)
+    gen = torch.Generator().manual_seed(n)
+    mask = torch.randint(0, 16, (n, 1), generator=gen, dtype=torch.int32) * (torch.rand(n, 1, generator=gen) < 0.3)
+    out = torch.arange(4 * n, dtype=torch.float32).view(n, 4)
+    kept = ((mask >> torch.arange(4)) & 1).bool()  # [n, 4]
+    total = int(kept.sum())
+    i64 = lambda k: torch.full((k,), -1, dtype=torch.int64, device="cuda")
+    counts, offsets = i64(n), i64(n + 1)
+    idx = torch.full((total,), -1, dtype=torch.int32, device="cuda")
+    w = torch.full((total,), -1.0, device="cuda")
+    ws = torch.empty(emr.compact_workspace_size(g, n), dtype=torch.uint8, device="cuda")
+    emr.compact(mask.cuda(), out.cuda(), g, n, idx, w, total, counts, offsets, ws)
+    c = kept.sum(1)
+    assert torch.equal(counts.cpu(), c)
+    assert torch.equal(offsets.cpu(), torch.cat([torch.zeros(1, dtype=torch.int64), c.cumsum(0)]))
+    pair, pos = kept.nonzero(as_tuple=True)
+    assert torch.equal(idx.cpu(), pos.int()) and torch.equal(w.cpu(), out[pair, pos])
+
+
+def test_segments_over_several_scan_ctas():
+    """1400 pairs of three segments: more segment counts than one CTA of the scan takes."""
+    kept, _ = compare(W.c2(D=8, P=350))
+    assert kept > 0
