@@ -313,8 +313,11 @@ emr_status emr_eval_filter(const void *pack_host, const emr_query *q, const emr_
 
 /* Bytes of device workspace emr_stream needs: the per-pair records, the
  * resident split plane (n_pairs x n_words x 4 bytes) and two chunk buffers
- * (band bits, tile flags, selection workspace and chunk_cap list entries each; the
- * kept weights are recomputed from the records, so no outputs are stored). */
+ * (band bits, tile flags, selection workspace and chunk_cap list entries each,
+ * flags and selection in the room of a second plane of the chunk and its
+ * compaction workspace, more than they use; the kept weights are recomputed from
+ * the records, so no outputs are stored). 5.3 GB for 16 genomes x 4 slots at depth
+ * 13 with chunks of 2^26 positions and 2^24 entries. */
 emr_status emr_stream_workspace_size(const void *pack_host, const emr_query *q, const emr_grid *grid,
                                      int64_t chunk_cap, size_t *bytes);
 
@@ -389,9 +392,10 @@ emr_status emr_stream_mode(const void *pack_host, const void *pack_dev, const em
  *    libemr's device code (and so the array) onto the device; make that first
  *    call before any stream capture.
  *  - All calls on a device share the one array and it keeps the previous
- *    call's contents. The one entry that must start at zero (the pair
- *    schedule's completion counter) is cleared by each call on its stream;
- *    every other entry is written before it is read. Calls whose work overlaps
+ *    call's contents. The entries that must start at zero (the pair
+ *    schedule's completion counter and, above 4096 pairs, its bin counts) are
+ *    cleared by each call on its stream; every other entry is written before
+ *    it is read. Calls whose work overlaps
  *    on the GPU (other streams, other host threads) race on the array:
  *    serialise them.
  * Errors: EMR_ERR_ARG, EMR_ERR_RANGE, EMR_ERR_CUDA. */
@@ -444,7 +448,8 @@ emr_status emr_eval_filter_tiles(const void *pack_host, const emr_query *q, cons
                                  uint8_t *tile_flags, void *ws, size_t ws_bytes, void *stream);
 
 /* Bytes of device workspace emr_select needs for n_pairs pairs (per pair and
- * dense tile: the tile's first list entry and a work item). */
+ * dense tile: the tile's first list entry and a work item; above 32 tiles, per pair
+ * and 32 tiles: a count and an offset). */
 emr_status emr_select_workspace_size(const emr_grid *grid, int32_t n_pairs, size_t *bytes);
 
 /* emr_mask_combine_types followed by emr_compact_records, computed only over the

@@ -111,7 +111,7 @@ def test_select_several_segments_per_pair():
 
 @pytest.mark.parametrize("P", [1, 255, 257, 2047, 2049, 5000])
 def test_offsets_are_the_scanned_counts(P):
-    """Around one count a thread (1024 pairs) and one pass (8192 pairs) of the scan, and several passes."""
+    """4 pairs up to 20000 (four slots a genome): one CTA of the scan (4096 counts) and several."""
     w = W.c2(D=2, P=P)
     dsc = emr.Discovery(w.pop, w.sources, w.D, w.theta, 0.1)
     dsc.run_discover()
